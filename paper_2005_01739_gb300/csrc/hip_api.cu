@@ -244,6 +244,7 @@ PmPairCat PmPlan::cat(char *b, int64_t N, double L, double R0, int los) const
     c.L = L;
     c.cs = L / n_c;
     c.wabs = (const double *)(b + o_zero) + 1;
+    c.err = err(b);
     c.G = (double *)(b + o_G);
     c.npairs = npairs(b);
     return c;
@@ -835,7 +836,7 @@ struct BkList {
 // Host copy of one catalog's a_lm-pass descriptor.
 template <typename T>
 static BkCat<T> bk_cat(char *b, double L, const BkList<T> &dl, const BkList<T> &rl, const int64_t *ranges,
-                       const double *k_edges, int n_k, double R0, double rand_weight, const double *S1,
+                       const double *k_edges, int n_k, double R0, double rand_weight, const double *S1, const int *err,
                        unsigned long long *npairs, double *cmom)
 {
     BkCat<T> a;
@@ -851,6 +852,7 @@ static BkCat<T> bk_cat(char *b, double L, const BkList<T> &dl, const BkList<T> &
     a.rcf = (const unsigned *)(b + rl.o_cf);
     a.shift = (const float2 *)(b + dl.o_shift);
     a.S1 = S1;
+    a.err = err;
     a.n_data = (int)N;
     a.n_rand = (int)N_r;
     a.dp0 = ranges ? ranges[0] : 0;
@@ -962,7 +964,7 @@ static hip_status bispec_impl(const float *pos, const float *w, int64_t N, const
     double *Wt = (double *)(b + o_wt), *DD = (double *)(b + o_dd);
     // S^a (the l = 0 data pair sum) comes from the a_lm pass; W~^a here
     if (!partial) HIP_CK(hip_window_transform(n_e, k_edges, R0, Wt, st), "window transform");
-    std::vector<BkCat<T>> cats(1, bk_cat<T>(b, L, dl, rl, ranges, k_edges, n_k, R0, -hS1 / (double)N_r, S1, npairs + 1,
+    std::vector<BkCat<T>> cats(1, bk_cat<T>(b, L, dl, rl, ranges, k_edges, n_k, R0, -hS1 / (double)N_r, S1, err, npairs + 1,
                                             (double *)(b + o_cmom)));
     cats[0].n_L = n_L;
     std::vector<BkHostCat> hc(1);
@@ -1215,7 +1217,7 @@ static hip_status bispec_batched_impl(const hip_bcatalog *cats, int nc, cudaStre
         // S^a comes from the a_lm pass; W~^a here
         HIP_CK(hip_window_transform(y.n_e, c.k_edges, c.R0, (double *)(b + y.o_wt), st), "window transform");
         bcats[i] = bk_cat<T>(b, c.L, y.dl, y.rl, nullptr, c.k_edges, c.n_k, c.R0, -hsm[(size_t)i * 9] / (double)c.N_r, small,
-                             npairs + 1, (double *)(b + y.o_cmom));
+                             (const int *)(small + 8), npairs + 1, (double *)(b + y.o_cmom));
         hcs[i] = BkHostCat{c.N + c.N_r, c.n_k, y.n_cc, c.R0, c.k_edges, (double *)(b + y.o_cmom),
                            (double *)(b + y.o_acc), c.N, (double *)(b + y.o_dd)};
     }
@@ -1351,7 +1353,7 @@ static hip_status bispec_analytic_impl(const float *pos, const float *w, int64_t
     // the data primaries' sum (no random primaries)
     BkList<T> none = dl;
     none.N = 0;
-    std::vector<BkCat<T>> cats(1, bk_cat<T>(b, L, dl, none, nullptr, k_edges, n_k, R0, 0.0, S1, npairs + 1,
+    std::vector<BkCat<T>> cats(1, bk_cat<T>(b, L, dl, none, nullptr, k_edges, n_k, R0, 0.0, S1, err, npairs + 1,
                                             (double *)(b + o_cmom)));
     std::vector<BkHostCat> hc(1);
     double *acc = (double *)(b + o_acc);

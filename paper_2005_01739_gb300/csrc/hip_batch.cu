@@ -244,6 +244,7 @@ static hip_status plan_build(hip_batch_plan *pl, cudaStream_t st)
                 m.L = c.L;
                 m.cs = c.L / L.n_c;
                 m.wabs = (const double *)(b + L.o_s1) + 2;
+                m.err = (const int *)(b + L.o_s1 + sizeof(double));
                 m.G = (double *)(b + L.o_G);
                 m.npairs = d.npairs;
                 hip_pm_items(m, hip_pm_warps());

@@ -57,6 +57,7 @@ struct BkCat {
     const unsigned *pcf, *rcf;
     const float2 *shift;
     const double *S1;
+    const int *err;            // the builds' error words (data, randoms): a rejected catalog is passed over
     double *S;
     int n_S;
 };

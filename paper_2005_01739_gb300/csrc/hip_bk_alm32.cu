@@ -366,6 +366,7 @@ __global__ void __launch_bounds__(NW * 32, 1)
     extern __shared__ __align__(16) unsigned char b32_raw[];
     __shared__ BkCat<float> a;
     __shared__ BkConst32 ks;
+    __shared__ int bad;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     BkWarp32 &sm = reinterpret_cast<BkWarp32 *>(b32_raw)[threadIdx.x >> 5];
     float *cm = reinterpret_cast<float *>(b32_raw + (blockDim.x >> 5) * sizeof(BkWarp32)) + (size_t)warp * words;
@@ -376,8 +377,17 @@ __global__ void __launch_bounds__(NW * 32, 1)
         for (int i = threadIdx.x; i < (int)(sizeof(a) / 4); i += blockDim.x)
             reinterpret_cast<int *>(&a)[i] = reinterpret_cast<const int *>(&cats[s.cat])[i];
         __syncthreads();
-        if (threadIdx.x == 0) bk32_const(ks, a);
+        if (threadIdx.x == 0) {
+            bk32_const(ks, a);
+            bad = a.err[0] | a.err[1];
+        }
         __syncthreads();
+        if (bad) {  // no primaries: the contraction passes over weights of zero
+            for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < s.g1 - s.g0; i += gridDim.x * blockDim.x)
+                spw[s.sp_off + i] = 0.0f;
+            __syncthreads();
+            continue;
+        }
         const BkConst32 k = ks;
         float2 kk[NCH], kl[NCH];
 #pragma unroll

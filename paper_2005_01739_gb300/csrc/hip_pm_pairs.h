@@ -33,7 +33,8 @@ struct PmFineBuf {
 };
 // Three launches.  S1 += sum of weights, wabs += sum of |weights| (both zero before;
 // N for unit weights), *err |= 1 on a non-finite position or weight (the particle
-// is then kept, in cell 0, so that the list stays well formed).
+// is then kept, in cell 0, so that the list stays well formed; the passes do not walk a
+// list whose error word is set: M such particles would be M^2 / 2 candidates).
 cudaError_t hip_build_fine(const float *pos, const float *w, int64_t N, double L, int n_c, int g, int64_t p0, int64_t p1,
                            const PmFineBuf &b, double *S1, double *wabs, int *err, cudaStream_t st);
 
@@ -65,6 +66,7 @@ struct PmPairCat {
     float R0, dc;
     double L, cs;          // box side, coarse cell side
     const double *wabs;    // sum |w|: sets the fixed-point unit
+    const int *err;        // the build's error word: a catalog it rejected is passed over
     double *G;             // [n_ell][Q][n_c S] FP64 totals (zero before the launch)
     unsigned long long *npairs;
     // work items: blocks of 32 sorted particles x n_col groups of neighbour columns x
