@@ -89,8 +89,8 @@ int hip_bk_intervals(double R0, double k_max)
     return q < 1.0 ? 1 : (int)q;
 }
 
-#define HIP_BK_WARPS 4
-#define HIP_BK_THREADS (HIP_BK_WARPS * 32)
+#define HIP_BK_WARPS 4  // most warps of a CTA
+#define HIP_BK_SMEM 232448  // opt-in shared memory of a CTA
 #define HIP_NLMP 36  // a drained pair's record: the 25 R_lm, w_j W, P_m(t) for m < HIP_BK64_M
 
 struct BkWarpSmem {
@@ -378,20 +378,20 @@ __device__ __forceinline__ void bk_primary(const BkCat<double> &a, int g, BkWarp
     }
 }
 
-// The a_lm pass: persistent CTAs of 4 warps; each warp takes work items (up to 8
+// The a_lm pass: persistent CTAs of up to 4 warps; each warp takes work items (up to 8
 // consecutive primaries of one span) from an atomic counter.  Per warp, the
 // C-term moments of the current catalog sit in a shared array, added to the warp's
 // slot after every item and to the catalog's moments when the warp leaves the catalog.
-__global__ void __launch_bounds__(HIP_BK_THREADS) k_bk_alm(const BkCat<double> *__restrict__ cats,
-                                                           const BkSpan *__restrict__ spans, int n_spans, int n_items,
-                                                           int ncc_max, double *__restrict__ X, double *__restrict__ sp,
-                                                           double *__restrict__ cm_slots, int *counter)
+__global__ void __launch_bounds__(HIP_BK_WARPS * 32) k_bk_alm(const BkCat<double> *__restrict__ cats,
+                                                              const BkSpan *__restrict__ spans, int n_spans, int n_items,
+                                                              int ncc_max, double *__restrict__ X, double *__restrict__ sp,
+                                                              double *__restrict__ cm_slots, int *counter)
 {
     extern __shared__ __align__(16) unsigned char bk_raw[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
     BkWarpSmem &sm = reinterpret_cast<BkWarpSmem *>(bk_raw)[warp];
-    double *cm = reinterpret_cast<double *>(bk_raw + HIP_BK_WARPS * sizeof(BkWarpSmem)) + (size_t)warp * ncc_max * HIP_BK_NM;
-    double *slot = cm_slots + ((size_t)blockIdx.x * HIP_BK_WARPS + warp) * ncc_max * HIP_BK_NM;
+    double *cm = reinterpret_cast<double *>(bk_raw + n_warps * sizeof(BkWarpSmem)) + (size_t)warp * ncc_max * HIP_BK_NM;
+    double *slot = cm_slots + ((size_t)blockIdx.x * n_warps + warp) * ncc_max * HIP_BK_NM;
     for (int i = lane; i < ncc_max * HIP_BK_NM; i += 32) cm[i] = 0.0;
     __syncwarp();
     BkEdges ed;
@@ -469,19 +469,23 @@ cudaError_t hip_bk_alm(const BkCat<double> *cats, const BkSpan *spans, int n_spa
                        double *X, double *sp, double *cm_slots, int *counter, cudaStream_t st)
 {
     if (nk_max > 31) return cudaErrorInvalidValue;
-    const size_t smem = HIP_BK_WARPS * (sizeof(BkWarpSmem) + sizeof(double) * (size_t)ncc_max * HIP_BK_NM);
+    // four warps, or as many as fit beside their C-term sums: four up to 149 intervals
+    // (R0 k_max 1192), one up to 830
+    const size_t per_warp = sizeof(BkWarpSmem) + sizeof(double) * (size_t)ncc_max * HIP_BK_NM;
+    const int warps = (int)std::max<size_t>(1, std::min<size_t>(HIP_BK_WARPS, HIP_BK_SMEM / per_warp));
+    const size_t smem = warps * per_warp;
     cudaError_t e = cudaFuncSetAttribute(k_bk_alm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = 0, nb = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_bk_alm, HIP_BK_THREADS, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_bk_alm, warps * 32, smem);
     if (nb < 1) nb = 1;
     if (nb > 16) nb = 16;
     int grid = sms * nb;
-    const int need = (n_items + HIP_BK_WARPS - 1) / HIP_BK_WARPS;
+    const int need = (n_items + warps - 1) / warps;
     if (grid > need) grid = need < 1 ? 1 : need;
-    k_bk_alm<<<grid, HIP_BK_THREADS, smem, st>>>(cats, spans, n_spans, n_items, ncc_max, X, sp, cm_slots, counter);
+    k_bk_alm<<<grid, warps * 32, smem, st>>>(cats, spans, n_spans, n_items, ncc_max, X, sp, cm_slots, counter);
     return cudaGetLastError();
 }
 
