@@ -514,7 +514,7 @@ extern "C" hip_status hip_power_from_pairs(const double *DD, int n_k, int ell_ma
 // at most `chunk` primaries, so X stays within HIP_BK_XBUDGET bytes.
 #define HIP_BK_XBUDGET ((size_t)8 << 30)  // a few percent of the 288 GB of HBM
 static int g_bk_tc_grid_cap = 0;  // tests: caps the contraction's CTAs (0 = one per SM)
-static int g_bk_chunk_cap = 0;    // tests: caps the primaries per chunk (0 = by the X budget)
+static int g_bk_chunk_cap = 0;    // tests: caps the primaries per chunk (0 = by the X budget), the FP64 tables at two
 static int g_bk_fold = 0;         // tests: primaries between the contraction's FP64 folds (0 = default)
 static int g_bk_cores = 0;        // tests: contract FP32 accumulators on the CUDA cores in FP64
 
@@ -537,7 +537,8 @@ struct BkPlan {
     long long chunk = 0;
     size_t o_cats = 0, o_spans = 0, o_segs = 0, o_X = 0, o_sp = 0, o_slots = 0, o_cc = 0, o_cnt = 0;
     size_t slots_bytes = 0;
-    size_t o_tab = 0, tab = 0;  // FP64: the catalogs' edge-function tables, `tab` doubles each
+    size_t o_tab = 0, tab = 0;  // FP64: n_tab edge-function tables of `tab` doubles, catalog i's at i mod n_tab
+    int n_tab = 0;              // most catalogs of a chunk
     bool tc = false;  // contraction on the tensor cores
 };
 
@@ -564,9 +565,14 @@ static BkPlan bk_plan(Carve &cv, int nc, int nk_max, int ncc_max, int n_L, doubl
     pl.slots_bytes = sizeof(T) == 4 ? hip_bk_alm32_slot_bytes(n_L * ncc_max * HIP_BK_NM) : hip_bk_alm_slot_bytes(ncc_max);
     pl.o_slots = cv.take(pl.slots_bytes);
     pl.n_L = n_L;
+    pl.n_tab = nc;
     if (sizeof(T) == 8) {
+        // the tables of one chunk's catalogs, within a budget like X's: all of 4096
+        // catalogs' at R0 k_max = 1200 and 31 bins would be 126 GB
         pl.tab = hip_bk_tab64_doubles(hip_bk_tab64_intervals(1.0, rk_max), nk_max + 1);
-        pl.o_tab = cv.take(sizeof(double) * pl.tab * nc);
+        pl.n_tab = (int)std::max<size_t>(1, std::min<size_t>(nc, HIP_BK_XBUDGET / (sizeof(double) * pl.tab)));
+        if (g_bk_chunk_cap > 0) pl.n_tab = std::min(pl.n_tab, 2);
+        pl.o_tab = cv.take(sizeof(double) * pl.tab * pl.n_tab);
     }
     pl.tc = sizeof(T) == 4 && hip_bk_tc_supported(nk_max);
     pl.o_cc = cv.take(cc_bytes);
@@ -632,16 +638,13 @@ static hip_status bk_run(std::vector<BkCat<T>> &cats, const std::vector<BkHostCa
         cats[i].S = hc[i].S;
         cats[i].n_S = hc[i].n_S;
         if (sizeof(T) == 8) {
-            cats[i].tab = (double *)(b + pl.o_tab) + pl.tab * i;
+            cats[i].tab = (double *)(b + pl.o_tab) + pl.tab * (i % pl.n_tab);
             cats[i].tab_n = hip_bk_tab64_intervals(hc[i].R0, hc[i].k_edges[hc[i].n_k]);
             cats[i].tab_scale = cats[i].tab_n / hc[i].R0;
         }
     }
     HIP_CK(cudaMemsetAsync(cnt, 0, sizeof(int) * 4, st), "memset");
     HIP_CK(cudaMemcpyAsync(dcats, cats.data(), sizeof(BkCat<T>) * nc, cudaMemcpyHostToDevice, st), "H2D catalogs");
-    if constexpr (sizeof(T) == 8)
-        for (int i = 0; i < nc; ++i)
-            HIP_CK(hip_bk_tab64(dcats, i, cats[i].tab_n, hc[i].n_k + 1, st), "edge-function table");
     const int P = hip_bk_tc_stage_prims(pl.nk_max);
     // optional event pairs around the stages: [chunk][a_lm, contraction], then the C terms
     std::vector<cudaEvent_t> evs;
@@ -660,12 +663,13 @@ static hip_status bk_run(std::vector<BkCat<T>> &cats, const std::vector<BkHostCa
     // walk the catalogs' primaries end to end, one chunk at a time
     int ci = 0;
     long long gi = 0;  // next primary of catalog ci
+    int n_tabbed = 0;  // FP64: catalogs whose table has been made
     while (ci < nc) {
         std::vector<BkSpan> spans;
         std::vector<BkSeg> segs;
         long long used = 0, x_off = 0, sp_off = 0;
         int items = 0, stages = 0;
-        while (ci < nc && used < pl.chunk) {
+        while (ci < nc && used < pl.chunk && (int)spans.size() < pl.n_tab) {
             const long long take = std::min(hc[ci].n_prim - gi, pl.chunk - used);
             if (take > 0) {
                 BkSpan s;
@@ -715,6 +719,9 @@ static hip_status bk_run(std::vector<BkCat<T>> &cats, const std::vector<BkHostCa
                                 pl.n_L * pl.ncc_max * HIP_BK_NM, slots, X, sp, cnt + 4, st),
                    "bispectrum a_lm pass");
         } else {
+            // tables of the catalogs that begin in this chunk, in the places of ones it does not reach
+            for (; n_tabbed <= spans.back().cat; ++n_tabbed)
+                HIP_CK(hip_bk_tab64(dcats, n_tabbed, cats[n_tabbed].tab_n, hc[n_tabbed].n_k + 1, st), "edge-function table");
             HIP_CK(cudaMemsetAsync(cnt, 0, sizeof(int), st), "memset");
             mark();
             HIP_CK(hip_bk_alm(dcats, dspans, (int)spans.size(), items, pl.nk_max, pl.ncc_max, X, sp, slots, cnt, st),
