@@ -385,7 +385,7 @@ def batched_summary(binding, stream, steps: int = 2, fp64: bool = True, bispectr
     res = plan.run(stream)
     default_shape = plan.shape()
     _, ms_default = replays()
-    # the autotuner's second stage (warps per CTA, fold period) on this batch, then the tuned plan is timed
+    # the autotuner's second stage (warps per CTA) on this batch, then the tuned plan is timed
     chosen, cand = plan.tune_kernel(stream)
     plan.run(stream)
     with ClockSampler(torch.cuda.current_device()) as clk:
@@ -395,13 +395,12 @@ def batched_summary(binding, stream, steps: int = 2, fp64: bool = True, bispectr
            "particles": int(sum(int(c["pos"].shape[0]) for c in cats)), "pair_bins": int(work),
            "value": work / (ms / 1e3), "unit": UNIT, "ms_per_replay": ms, "launches_per_replay": plan.launches,
            "clocks": clk.summary(),
-           "autotune": {"shape": dict(zip(("particles_per_cell", "warps_per_cta", "fold_pairs"), plan.shape())),
-                        "default_shape": dict(zip(("particles_per_cell", "warps_per_cta", "fold_pairs"),
-                                                  default_shape)),
+           "autotune": {"shape": dict(zip(("particles_per_cell", "warps"), plan.shape())),
+                        "default_shape": dict(zip(("particles_per_cell", "warps"), default_shape)),
                         "default_ms_per_replay": ms_default,
-                        "candidates_ms": {f"warps{w}_fold{f}": v for (w, f), v in cand.items()},
+                        "candidates_ms": {f"warps{w}": v for (w, _), v in cand.items()},
                         "note": "ms_per_replay is the tuned plan (hip_batch_plan_tune_kernel at the default 64 "
-                                "particles per cell); warps 0 / fold 0 = the defaults (by occupancy / 16384)"}}
+                                "particles per cell); warps 4 / 8 are 16 / 28 warps per CTA, 0 = the default 28"}}
     mixed = [(np.array(P), np.array(DD)) for P, DD, _ in res]
     plan.close()
     if fp64:

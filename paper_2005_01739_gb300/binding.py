@@ -331,9 +331,11 @@ class BatchPlan:
         return int(chosen.value), dict(zip((4, 8, 16, 32, 64, 128, 256, 0), (float(x) for x in ms)))
 
     def tune_kernel(self, stream=None):
-        """Autotune the moment pass's warps per CTA and fold period at the plan's cell
-        occupancy (hip_batch_plan_tune_kernel): returns ((warps, fold) chosen,
-        {(warps, fold): replay ms})."""
+        """Autotune the moment pass's warps per CTA at the plan's cell occupancy
+        (hip_batch_plan_tune_kernel): returns ((warps, fold) chosen, {(warps, fold):
+        replay ms}).  warps 4 and 8 are the FP64 pass's warps per CTA and stand for 16
+        and 28 in mixed precision; the fold has no effect (16384 is reported, and the
+        three folds of a warps setting share one time)."""
         w, f = ctypes.c_int(0), ctypes.c_int(0)
         ms = (ctypes.c_float * 6)()
         rc = self._lib.hip_batch_plan_tune_kernel(self._plan, _stream_handle(stream), ctypes.byref(w), ctypes.byref(f),
@@ -345,7 +347,8 @@ class BatchPlan:
         return (int(w.value), int(f.value)), dict(zip(shapes, (float(x) for x in ms)))
 
     def shape(self):
-        """(occ, warps, fold) of the plan (warps 0 = by occupancy, fold 0 = 16384)."""
+        """(occ, warps, fold) of the plan (warps 0 = a new plan's: by occupancy in FP64, 28
+        in mixed precision; the fold has no effect)."""
         o, w, f = ctypes.c_int(0), ctypes.c_int(0), ctypes.c_int(0)
         self._lib.hip_batch_plan_shape(self._plan, ctypes.byref(o), ctypes.byref(w), ctypes.byref(f))
         return int(o.value), int(w.value), int(f.value)

@@ -78,8 +78,9 @@ struct hip_batch_plan {
     cudaStream_t cap_stream = nullptr;
     int launches = 0;
     int occ = 64;   // target particles per cell (see batch_cells_per_side)
-    int warps = 0;  // moment pass: warps per CTA (4 or 8; 0 = by the cell occupancy)
-    int fold = 0;   // as set by the autotuner (the FP32 sums need no folds: see hip_pm_pairs.cu)
+    int warps = 0;  // moment pass, as set by the autotuner: 4 or 8 (FP64: warps per CTA, 0 = by the cell
+                    // occupancy; mixed: 16 or 28 warps per CTA, 0 = 28)
+    int fold = 0;   // as reported by the autotuner (neither precision folds: see hip_pm_pairs.cu)
 };
 
 extern "C" const char *hip_batch_message(void) { return g_batch_msg; }
@@ -572,10 +573,12 @@ extern "C" hip_status hip_batch_plan_tune(hip_batch_plan *pl, void *cuda_stream,
     return HIP_OK;
 }
 
-// The in-kernel shapes of the moment pass at the plan's cell occupancy: warps per
-// CTA x fold period, each candidate timed on one replay after a warm-up.
+// The in-kernel shapes of the moment pass at the plan's cell occupancy: two settings of
+// the warps per CTA, each timed on one replay after a warm-up.  Of the interface's six
+// (warps, fold) entries the three folds of a setting are one shape and one time.
 static const int k_tune_warps[] = {4, 8};
-static const int k_tune_fold[] = {4096, 8192, 16384};
+#define HIP_TUNE_FOLDS 3
+#define HIP_TUNE_FOLD 16384  // the fold reported
 
 extern "C" hip_status hip_batch_plan_tune_kernel(hip_batch_plan *pl, void *cuda_stream, int *warps_out, int *fold_out,
                                                  float *ms_out)
@@ -584,29 +587,26 @@ extern "C" hip_status hip_batch_plan_tune_kernel(hip_batch_plan *pl, void *cuda_
     if (!pl) return HIP_ERR_ARG;
     std::lock_guard<std::mutex> lk(hip_api_mutex());
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    int best_w = 0, best_f = 0, i = 0;
+    int best_w = 0, i = 0;
     float best_ms = 0.0f;
-    for (int w : k_tune_warps)
-        for (int f : k_tune_fold) {
-            plan_release(pl);
-            pl->warps = w;
-            pl->fold = f;
-            hip_status hs = pl->prec == HIP_PREC_MIXED ? plan_build<float>(pl, st) : plan_build<double>(pl, st);
-            if (hs == HIP_OK) hs = plan_run_locked(pl, st, nullptr);  // warm-up
-            float ms = 0.0f;
-            if (hs == HIP_OK) hs = plan_run_locked(pl, st, &ms);
-            if (hs != HIP_OK) return hs;
+    for (int w : k_tune_warps) {
+        plan_release(pl);
+        pl->warps = w;
+        hip_status hs = pl->prec == HIP_PREC_MIXED ? plan_build<float>(pl, st) : plan_build<double>(pl, st);
+        if (hs == HIP_OK) hs = plan_run_locked(pl, st, nullptr);  // warm-up
+        float ms = 0.0f;
+        if (hs == HIP_OK) hs = plan_run_locked(pl, st, &ms);
+        if (hs != HIP_OK) return hs;
+        for (int f = 0; f < HIP_TUNE_FOLDS; ++f, ++i)
             if (ms_out) ms_out[i] = ms;
-            ++i;
-            if (best_w == 0 || ms < best_ms) {
-                best_w = w;
-                best_f = f;
-                best_ms = ms;
-            }
+        if (best_w == 0 || ms < best_ms) {
+            best_w = w;
+            best_ms = ms;
         }
+    }
     plan_release(pl);
     pl->warps = best_w;
-    pl->fold = best_f;
+    pl->fold = HIP_TUNE_FOLD;
     hip_status hs = pl->prec == HIP_PREC_MIXED ? plan_build<float>(pl, st) : plan_build<double>(pl, st);
     if (hs != HIP_OK) return hs;
     if (warps_out) *warps_out = pl->warps;

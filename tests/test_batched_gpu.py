@@ -162,3 +162,18 @@ def test_plan_autotune_keeps_results():
             assert abs(n1 - n0) <= max(2, int(2e-6 * n0))
     finally:
         plan.close()
+
+
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+def test_kernel_tuner_times_each_shape_once(prec):
+    # the fold has no effect: the three folds of a warps setting are one shape with one
+    # time, and the fold reported does not depend on timing noise
+    plan = binding.BatchPlan([c for c, _, _ in _batch(True)], prec)
+    try:
+        (w, f), ms = plan.tune_kernel()
+        assert f == 16384
+        for q in (4, 8):
+            assert len({ms[q, g] for g in (4096, 8192, 16384)}) == 1
+        assert ms[w, f] == min(ms.values())
+    finally:
+        plan.close()
