@@ -322,13 +322,12 @@ const char *hip_batch_message(void);
  * but all scratch lives in one statically sized device array of
  * hip_noalloc_capacity() bytes (64 MiB) that every device loading the library
  * reserves until the process exits; no cudaMalloc/cudaFree or other allocating
- * routine is called.  It is for callers that cannot allocate device memory
+ * routine is called, on the device or on the host.  It is for callers that cannot allocate device memory
  * while they run: a host application whose own memory pool has already
  * reserved the device's memory (a library cudaMalloc would fail or take memory
  * the pool counts on), or a service that must know its peak device footprint
- * before it starts.  The call is eager and synchronising, like hip_power: it
- * reads an error word back to the host after the cell build and synchronises
- * `cuda_stream` before returning.
+ * before it starts.  The call is eager and synchronises `cuda_stream` before
+ * returning, like hip_power.
  *
  * Limit: the call needs about 24 bytes per particle for device-resident inputs
  * (36 for host positions, 40 with host weights), plus cell tables and per-CTA partial sums; a call that

@@ -8,9 +8,11 @@
 // counts on), and services that must know their peak device footprint before
 // they start, so that no call may grow it.
 //
-// The call is eager and synchronising: it reads the cell build's error word back
-// to the host in the middle of the call and synchronises `cuda_stream` before it
-// returns, like hip_power.
+// The call allocates no host memory either: its results pass through a fixed array.
+//
+// The call is eager and synchronises `cuda_stream` before it returns, like hip_power.
+// The moment pass's error word comes back with its results; the direct pass reads it
+// after the cell build, in the middle of the call.
 //
 // The array below is reserved on every device that loads this library, for the
 // lifetime of the process.  Its device address is looked up once per device
@@ -26,7 +28,6 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
-#include <vector>
 
 #include "hip_internal.h"
 #include "hip_moments.h"
@@ -37,6 +38,7 @@
 static __device__ __align__(256) unsigned char g_noalloc_scratch[HIP_NOALLOC_BYTES];
 static void *g_noalloc_ptr[64];
 static char g_noalloc_msg[256];
+static double g_noalloc_out[2 * 3 * HIP_MAX_BINS + 2];  // results of a call (PmFinish::out), under the API mutex
 
 std::mutex &hip_api_mutex();
 
@@ -133,11 +135,10 @@ extern "C" hip_status hip_power_noalloc(const float *pos, const float *w, int64_
         HIP_NA_CK(pl.build(b, dposp, dwp, N, L, prim_begin, prim_end, st), "cell build");
         HIP_NA_CK(pl.pairs(b, N, L, R0, los_axis, prim_begin == 0 && prim_end == N, st), "moment pass");
         HIP_NA_CK(pl.finish(b, L, R0, k_edges, st), "finalize");
-        std::vector<double> h(pl.out_doubles());
-        HIP_NA_CK(cudaMemcpyAsync(h.data(), pl.out(b), sizeof(double) * h.size(), cudaMemcpyDeviceToHost, st),
+        HIP_NA_CK(cudaMemcpyAsync(g_noalloc_out, pl.out(b), sizeof(double) * pl.out_doubles(), cudaMemcpyDeviceToHost, st),
                   "D2H results");
         HIP_NA_CK(cudaStreamSynchronize(st), "stream sync");
-        return hip_pm_unpack(h.data(), n_ell * n_k, P_out, DD_out, npairs_out);
+        return hip_pm_unpack(g_noalloc_out, n_ell * n_k, P_out, DD_out, npairs_out);
     }
     double *small = (double *)(b + o_small);
     double *S1 = small;

@@ -172,3 +172,16 @@ def test_window_omega_argument_checks(lib):
         with pytest.raises(binding.HipError) as ei:
             binding.hip_window_omega(*args)
         assert ei.value.status == code
+
+
+def test_noalloc_entry_allocates_no_host_memory(lib):
+    # hip_power_noalloc promises that no allocating routine is called: its object refers to
+    # neither operator new nor malloc
+    import shutil
+    import subprocess
+    obj = os.path.join(build.OUT, "hip_noalloc.cu.o")
+    if not shutil.which("nm") or not os.path.exists(obj):
+        pytest.skip("no nm or object file")
+    names = subprocess.run(["nm", "-u", obj], capture_output=True, text=True, check=True).stdout.split()
+    assert "cudaMemcpyAsync" in names
+    assert not [n for n in names if n.startswith(("_Zn", "_Zd")) or n in ("malloc", "calloc", "realloc")], names
