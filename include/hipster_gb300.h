@@ -40,10 +40,12 @@ typedef enum {
 typedef enum { HIP_WINDOW_PHILCOX = 0 } hip_window;
 
 /* Arithmetic of the pair kernels.  FP64: every per-pair and per-bin quantity in
- * double precision (the plain baseline).  MIXED: pair geometry, bin-averaged
- * Bessel functions and per-warp (moment pass: per-CTA) accumulation in FP32,
- * folded into FP64 every few ten thousand pairs; cross-warp reduction,
- * normalisation and the analytic random-pair terms in FP64. */
+ * double precision (the plain baseline).  MIXED: pair geometry and bin-averaged
+ * Bessel functions in FP32; the power spectrum's moment pass rounds each pair's
+ * terms once to fixed-point words whose sums are exact, the other passes
+ * accumulate per warp in FP32 and fold into FP64 (after 64 pairs at most, or per
+ * primary); cross-warp reduction, normalisation and the analytic random-pair
+ * terms in FP64. */
 typedef enum { HIP_PREC_FP64 = 0, HIP_PREC_MIXED = 1 } hip_precision;
 
 #define HIP_MAX_BINS 255

@@ -550,14 +550,15 @@ def debug_Fb(l: int, u: float) -> float:
 
 def debug_bk_caps(tc_grid_cap: int = 0, chunk_cap: int = 0) -> None:
     """Test hook: cap the CTAs of the bispectrum's tensor-core contraction and the
-    primaries per chunk of the bispectrum pass (0 = the library's own choice)."""
+    primaries per chunk of the bispectrum pass (0 = the library's own choice; a cap
+    also leaves the FP64 pass two places for edge-function tables)."""
     load().hip_debug_bk_caps(int(tc_grid_cap), int(chunk_cap))
 
 
 def debug_bk_mode(contract_on_cores: bool = False, fold_prims: int = 0) -> None:
     """Test hook: contract the mixed path's accumulators on the CUDA cores in FP64
-    instead of the tensor cores, and/or set the primaries between the tensor-core
-    contraction's FP64 folds (0 = the library's default)."""
+    instead of the tensor cores.  fold_prims has no effect (the tensor-core
+    contraction folds after every unit of work)."""
     load().hip_debug_bk_mode(int(bool(contract_on_cores)), int(fold_prims))
 
 

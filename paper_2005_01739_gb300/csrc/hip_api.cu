@@ -515,7 +515,6 @@ extern "C" hip_status hip_power_from_pairs(const double *DD, int n_k, int ell_ma
 #define HIP_BK_XBUDGET ((size_t)8 << 30)  // a few percent of the 288 GB of HBM
 static int g_bk_tc_grid_cap = 0;  // tests: caps the contraction's CTAs (0 = one per SM)
 static int g_bk_chunk_cap = 0;    // tests: caps the primaries per chunk (0 = by the X budget), the FP64 tables at two
-static int g_bk_fold = 0;         // tests: primaries between the contraction's FP64 folds (0 = default)
 static int g_bk_cores = 0;        // tests: contract FP32 accumulators on the CUDA cores in FP64
 
 // Stage timing of the last bispectrum primary sum (when profiling is on): the
@@ -731,8 +730,7 @@ static hip_status bk_run(std::vector<BkCat<T>> &cats, const std::vector<BkHostCa
         if (hc[0].G)  // anisotropic: the matching-m Gram blocks (every catalog of the call is anisotropic)
             HIP_CK(hip_bk_aniso_gram(dsegs, (int)segs.size(), pl.nk_max, used, st), "anisotropic Gram");
         else if (pl.tc && !g_bk_cores)
-            HIP_CK(hip_bk_contract_tc(dsegs, (int)segs.size(), stages, pl.nk_max, cnt + 1, g_bk_tc_grid_cap, g_bk_fold,
-                                      st),
+            HIP_CK(hip_bk_contract_tc(dsegs, (int)segs.size(), stages, pl.nk_max, cnt + 1, g_bk_tc_grid_cap, st),
                    "bispectrum contraction (tensor cores)");
         else
             HIP_CK(hip_bk_contract_f64<T>(dsegs, (int)segs.size(), used, pl.nk_max, st), "bispectrum contraction");
@@ -893,10 +891,10 @@ extern "C" void hip_debug_bk_caps(int tc_grid_cap, int chunk_cap)
     g_bk_chunk_cap = chunk_cap > 0 ? chunk_cap : 0;
 }
 
-extern "C" void hip_debug_bk_mode(int contract_on_cores, int fold_prims)
+// The second argument has no effect: the contraction folds after every unit.
+extern "C" void hip_debug_bk_mode(int contract_on_cores, int)
 {
     g_bk_cores = contract_on_cores != 0;
-    g_bk_fold = fold_prims > 0 ? fold_prims : 0;
 }
 
 template <typename T>

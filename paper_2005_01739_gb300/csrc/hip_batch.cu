@@ -144,8 +144,10 @@ static hip_status plan_build(hip_batch_plan *pl, cudaStream_t st)
         L.o_cid = cv.take(sizeof(int) * N);
         L.o_start = cv.take(sizeof(int) * (cells + 1));
         L.o_acc = cv.take(sizeof(double) * 3 * L.n_e);
-        L.o_s1 = cv.take(sizeof(double) * 3);  // S1, error word, sum |w|
-        L.o_np = cv.take(sizeof(unsigned long long));
+        if (!pm32) {
+            L.o_s1 = cv.take(sizeof(double) * 2);  // S1, error word
+            L.o_np = cv.take(sizeof(unsigned long long));
+        }
         L.o_wt = cv.take(sizeof(double) * c.n_k);
         L.o_dd = cv.take(sizeof(double) * 3 * c.n_k);
         L.o_p = cv.take(sizeof(double) * 3 * c.n_k);
@@ -164,7 +166,7 @@ static hip_status plan_build(hip_batch_plan *pl, cudaStream_t st)
         const size_t nf = (size_t)L.n_c * L.g;
         L.o_fill = cv.take(sizeof(int) * nf * nf * nf);
         L.o_col = cv.take(sizeof(int) * nf * nf);
-        L.o_s1 = cv.take(sizeof(double) * 3);
+        L.o_s1 = cv.take(sizeof(double) * 3);  // S1, error word, sum |w|
         L.o_np = cv.take(sizeof(unsigned long long));
         L.o_G = cv.take(sizeof(double) * 3 * sp.Q * (size_t)L.pm_nc * sp.S);
     }
@@ -194,8 +196,9 @@ static hip_status plan_build(hip_batch_plan *pl, cudaStream_t st)
         const CatLayout &L = pl->lay[i];
         BatchCat<T> &d = bc[oi];
         std::memset(&d, 0, sizeof(d));
-        d.cl = CellList<T>{(T *)(b + L.o_x), (T *)(b + L.o_y), (T *)(b + L.o_z), (float *)(b + L.o_ws),
-                           (int *)(b + L.o_idx), (int *)(b + L.o_start), L.n_c, c.L, c.L / L.n_c};
+        if (!pm32)
+            d.cl = CellList<T>{(T *)(b + L.o_x), (T *)(b + L.o_y), (T *)(b + L.o_z), (float *)(b + L.o_ws),
+                               (int *)(b + L.o_idx), (int *)(b + L.o_start), L.n_c, c.L, c.L / L.n_c};
         d.p0 = c.prim_begin;
         d.p1 = c.prim_end;
         d.los = c.los_axis;

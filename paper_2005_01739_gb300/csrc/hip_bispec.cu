@@ -95,7 +95,7 @@ int hip_bk_intervals(double R0, double k_max)
 
 struct BkWarpSmem {
     alignas(16) double qa[64][4];            // accepted neighbours: primary minus neighbour, w_j
-    alignas(16) double qd[32][HIP_NLMP];     // drained pairs: R_lm (0..24), r (25), w_j W (26)
+    alignas(16) double qd[32][HIP_NLMP];     // drained pairs: R_lm (0..24), w_j W (25), P_m(t) (26 + m)
     double pt[32][HIP_BK_NM + 1];            // C-term weight s_p w_j^2 W^2 times R_m(t), m < 32
     int tc[32];                         // table interval of each drained pair
     int qc[32];                         // C-term interval of each drained pair
@@ -115,11 +115,14 @@ cudaError_t hip_sorted_cells(const int *cell_start, int n_cells, int *scell, cud
 }
 
 // Edge functions of the FP64 pass: F_l(k_e r) as Legendre series in r on intervals
-// with k_max h <= 1/4 (band-limited: the first neglected term, (1/4)^10 / 19!!, is
-// 1.5e-15), tabulated per call as tab[interval][m][l][edge].  Evaluating them per
+// with k_max h <= 1/4 (band-limited: the first neglected term is at most (1/4)^10 / 19!! =
+// 1.5e-15, and about 1e-17 with F_l's own spectrum), tabulated as
+// tab[interval][m][l][edge] for the catalogs of a chunk.  Evaluating them per
 // (pair, edge) (sine, cosine and the sine integral's three ranges, all run by a warp
 // whose lanes are the edges) took about 235 FP64 operations; the series take 50, and
 // the table's own 12 evaluations per (interval, edge) are a fraction of a millisecond.
+// Error against 64 bits (2-norm, median of 24 catalogs) by evaluation / so: 1.2e4 data
+// particles 1.28e-15 / 1.26e-15, 1500 1.49e-15 / 1.48e-15.
 #define HIP_BK64_NG 12
 #define HIP_BK64_CB 8
 static __constant__ double c_t64_x[HIP_BK64_NG], c_t64_P[HIP_BK64_NG][HIP_BK64_M];  // nodes; w_g (2m+1)/2 P_m

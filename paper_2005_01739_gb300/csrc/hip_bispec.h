@@ -116,14 +116,15 @@ int hip_bk_tc_stage_prims(int nk_max);
 // Sum_p s_p X_p X_p^T over the segments (device-resident table) on the tensor
 // cores (tcgen05.mma kind::f16 on an exact three-slice BF16 split of X, the six
 // slice products in three FP32 TMEM accumulators that stay exact, folded into
-// float-float rows every fold_prims primaries, 0 = every stage, and into FP64).
+// float-float sums after every unit and into FP64 at the end of a catalog).
 // n_stages: total stages of all segments; status: device int, bit 0 set if a
 // bounded wait gave up (the results are then invalid).  max_grid caps the CTAs
 // (tests).  Supported for n_k <= 63 (hip_bk_tc_supported).
 bool hip_bk_tc_supported(int nk_max);
 cudaError_t hip_bk_contract_tc(const BkSeg *segs, int n_segs, int n_stages, int nk_max, int *status, int max_grid,
-                               int fold_prims, cudaStream_t st);
-// The same contraction in FP64 on the CUDA cores (plain path; T = the type of X):
+                               cudaStream_t st);
+// The same contraction in FP64 on the CUDA cores (T = the type of X: double for the plain
+// path; float only through hip_debug_bk_mode, the tests' check of the tensor cores):
 // the segments' primaries (n_total of them) laid end to end.
 template <typename T>
 cudaError_t hip_bk_contract_f64(const BkSeg *segs, int n_segs, long long n_total, int nk_max, cudaStream_t st);

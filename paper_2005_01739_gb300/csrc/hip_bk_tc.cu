@@ -29,8 +29,8 @@
 //     A0 = h h^T,  A1 = h m^T + m h^T,  A2 = h l^T + l h^T + m m^T
 // (separate tensor-memory columns; the dropped terms are below 2^-32 of A0) are
 // exact whatever the accumulator's rounding (kind::f16, BF16 operands, FP32
-// accumulation); they are added in FP64 into the CTA's rows in shared memory
-// after every unit of work.  Primary weights enter as sqrt|s_p| before the split
+// accumulation); after every unit of work they are added to the CTA's sums in shared
+// memory, each an unevaluated sum of two floats (about 48 bits).  Primary weights enter as sqrt|s_p| before the split
 // and the sign through the MMA's negate-A bit, so a unit holds primaries of one
 // sign (a stage with both signs is issued twice, once per sign, with the other
 // primaries zeroed).
@@ -44,9 +44,8 @@
 // unit u + 1 into the second slice buffer while the MMAs of unit u run; one
 // thread issues the MMAs and commits them to an mbarrier; the warps read the
 // accumulators back with tcgen05.ld (warp w owns lanes 32 (w mod 4)..+31, the
-// four warps of a lane group split the columns) and add them to the CTA's FP64
-// rows, which go to the catalog's FP64 sums (atomics) when the CTA leaves the
-// catalog.  Every wait is bounded (about two seconds); a wait that gives up sets
+// four warps of a lane group split the columns) and add them to the CTA's sums,
+// which go to the catalog's FP64 sums (atomics) when the CTA leaves the catalog.  Every wait is bounded (about two seconds); a wait that gives up sets
 // bit 0 of *status, stops the CTA's work, and the CTA still waits (bounded) for
 // its own MMAs before it frees its tensor memory.
 #include <cstdint>
@@ -152,7 +151,7 @@ static int tc_tiles(int nk)
 
 // Byte offsets of the dynamic shared memory (from the 1024-byte aligned base):
 // two buffers of the three slices of one tile, two staging buffers of a stage's
-// X block, the rows as two float arrays, three mbarriers.  The same function
+// X block, the sums as float pairs, three mbarriers.  The same function
 // lays out the kernel and sizes (and checks) the launch.
 struct TcLayout {
     size_t slice;     // bytes of one slice operand (128 rows x K bf16)
@@ -404,9 +403,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, 1));
         vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, 2));
         // 2^e > vmax, from the exponent field (vmax = f 2^e with f in [0.5, 1)):
-        // x 2^-e in (-1, 1); e is clamped so that both powers of two are normal
+        // x 2^-e in (-1, 1); e is clamped so that the powers of two below are normal.
+        // A row above 2^110 would be cut wrongly, but its own product in A0 leaves
+        // FP32's range from 2^64 on
         int e = vmax > 0.f ? (int)((__float_as_uint(vmax) >> 23) & 0xFFu) - 126 : 0;
-        e = e < -100 ? -100 : (e > 110 ? 110 : e);  // all powers of two below are normal
+        e = e < -100 ? -100 : (e > 110 ? 110 : e);
         // slices by adding and subtracting 1.5 2^23 units, units 2^(e-8), 2^(e-16),
         // 2^(e-24): each rounds to the nearest multiple exactly as an integer rounding
         // of the scaled value, without scaling; every slice is exact in BF16, whose
@@ -476,7 +477,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         }
         asm volatile("tcgen05.fence::after_thread_sync;");
     };
-    // A0 + A1 + A2 of unit u -> the CTA's FP64 rows (the unit's MMAs are done)
+    // A0 + A1 + A2 of unit u -> the CTA's sums (the unit's MMAs are done)
     auto fold = [&](const TcUnit &u) {
         const TcGeom &g = s_geo[u.slot];
         const short *lar = s_row[u.slot][u.t];
@@ -525,7 +526,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         }
         asm volatile("tcgen05.fence::before_thread_sync;");
     };
-    // this CTA's rows -> the segment's FP64 accumulator
+    // this CTA's sums -> the segment's FP64 accumulator
     auto flush = [&](int si) {
         __syncthreads();
         const BkSeg &sg = SEG(si);
@@ -597,9 +598,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 }
 
 cudaError_t hip_bk_contract_tc(const BkSeg *segs, int n_segs, int n_stages, int nk_max, int *status, int max_grid,
-                               int fold_prims, cudaStream_t st)
+                               cudaStream_t st)
 {
-    (void)fold_prims;  // the exact split folds after every unit
     if (!hip_bk_tc_supported(nk_max)) return cudaErrorInvalidValue;
     if (n_stages < 1) return cudaSuccess;
     const int P = hip_bk_tc_stage_prims(nk_max);

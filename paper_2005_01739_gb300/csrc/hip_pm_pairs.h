@@ -42,8 +42,9 @@ cudaError_t hip_build_fine(const float *pos, const float *w, int64_t N, double L
 // sub-interval of half-width h, k h <= 2 / S, and the first neglected Legendre
 // term of an edge function is (k h)^Q / (2Q - 1)!! of it: 9.1e-9 (S = 64, Q = 4),
 // 1.0e-9 (32, 5), 3.7e-10 (16, 6), 4.5e-10 (8, 7), below the FP32 rounding of a pair's term (6e-8)
-// and of varying sign from pair to pair.  The widest S whose words fit one CTA's
-// shared memory is taken: fewer atomics per pair.
+// and of varying sign from pair to pair.  The widest S whose words for three multipoles
+// fit one CTA's shared memory is taken: fewer atomics per pair.  (One or two multipoles
+// would fit wider ones beyond these lines; they take the same.)
 struct PmSplit {
     int S, Q;
 };
