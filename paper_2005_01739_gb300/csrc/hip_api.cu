@@ -227,7 +227,7 @@ cudaError_t PmPlan::build(char *b, const float *pos, const float *w, int64_t N, 
     if (e != cudaSuccess) return e;
     const PmFineBuf fb{(int *)(b + o_fill), (int *)(b + o_col),    (int *)(b + o_start),   (int *)(b + o_cid),
                        (float4 *)(b + o_p4), (unsigned *)(b + o_cf), (float2 *)(b + o_shift),
-                       f64 ? (double *)(b + o_x64) : nullptr};
+                       f64 ? (double *)(b + o_x64) : nullptr, err(b) + 1};
     double *z = (double *)(b + o_zero);
     return hip_build_fine(pos, w, N, L, n_c, g, p0, p1, fb, z, z + 1, err(b), st);
 }
@@ -244,7 +244,6 @@ PmPairCat PmPlan::cat(char *b, int64_t N, double L, double R0, int los) const
     c.L = L;
     c.cs = L / n_c;
     c.wabs = (const double *)(b + o_zero) + 1;
-    c.err = err(b);
     c.G = (double *)(b + o_G);
     c.npairs = npairs(b);
     return c;

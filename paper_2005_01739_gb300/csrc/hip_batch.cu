@@ -248,7 +248,6 @@ static hip_status plan_build(hip_batch_plan *pl, cudaStream_t st)
                 m.L = c.L;
                 m.cs = c.L / L.n_c;
                 m.wabs = (const double *)(b + L.o_s1) + 2;
-                m.err = (const int *)(b + L.o_s1 + sizeof(double));
                 m.G = (double *)(b + L.o_G);
                 m.npairs = d.npairs;
                 hip_pm_items(m, hip_pm_warps());
@@ -330,6 +329,8 @@ static hip_status plan_build(hip_batch_plan *pl, cudaStream_t st)
         return HIP_ERR_CUDA;
     }
     int launches = 0;
+    std::vector<int> place(nc);  // of a catalog in the launch's order
+    for (int oi = 0; oi < nc; ++oi) place[order[oi]] = oi;
     cudaError_t ce = cudaMemsetAsync(err, 0, sizeof(int) * 4, st);  // the work counter
     if (pm32 && ce == cudaSuccess) ce = cudaMemsetAsync(b + o_zero, 0, zero_bytes, st);
     for (int i = 0; i < nc && ce == cudaSuccess; ++i) {
@@ -340,7 +341,8 @@ static hip_status plan_build(hip_batch_plan *pl, cudaStream_t st)
         launches += 3;
         if (pm32) {
             const PmFineBuf fb{(int *)(b + L.o_fill), (int *)(b + L.o_col), (int *)(b + L.o_start), (int *)(b + L.o_cid),
-                               (float4 *)(b + L.o_p4), (unsigned *)(b + L.o_cf), (float2 *)(b + L.o_shift)};
+                               (float4 *)(b + L.o_p4), (unsigned *)(b + L.o_cf), (float2 *)(b + L.o_shift), nullptr,
+                               (int *)(b + o_cnt) + place[i]};
             double *s1 = (double *)(b + L.o_s1);
             ce = hip_build_fine(pos, w, c.N, c.L, L.n_c, L.g, c.prim_begin, c.prim_end, fb, s1, s1 + 2, (int *)(s1 + 1), st);
             continue;

@@ -399,7 +399,6 @@ template <int MASK, bool FULL>
 __global__ void __launch_bounds__(HIP_PM64_WARPS * 32, 3)
     k_power_moments(const __grid_constant__ PmPairCat cat, const double *__restrict__ x64, double R0, double dc, int *counter)
 {
-    if (__ldg(cat.err)) return;  // uniform
     extern __shared__ __align__(16) unsigned char pm_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_c = cat.n_c, n_cp = n_c | 1;
     PmRows &rows = reinterpret_cast<PmRows *>(pm_raw)[warp];

@@ -19,6 +19,7 @@ struct PmFine {
 };
 
 #define HIP_PM_FINE_MAX (1 << 24)  // most fine cells of a list
+#define HIP_PM_NO_ITEMS (1 << 30)  // more than any catalog's items
 // Fine cells per coarse cell and axis.
 int hip_pm_fine_grid(int64_t N, int n_c, int64_t max_cells);
 // Scratch of a build that must be zero before it: int fill[n_f^3], col[n_f^2];
@@ -30,11 +31,12 @@ struct PmFineBuf {
     unsigned *cf;
     float2 *shift;
     double *x64 = nullptr;  // FP64 pass: [N][3] sorted positions, wrapped into the box
+    int *counter = nullptr;  // the moment passes' work counter (zero before), HIP_PM_NO_ITEMS on a rejected catalog
 };
 // Three launches.  S1 += sum of weights, wabs += sum of |weights| (both zero before;
 // N for unit weights), *err |= 1 on a non-finite position or weight (the particle
-// is then kept, in cell 0, so that the list stays well formed; the passes do not walk a
-// list whose error word is set: M such particles would be M^2 / 2 candidates).
+// is then kept, in cell 0, so that the list stays well formed; M such particles would be
+// M^2 / 2 candidates, so the work counter is moved past every item and no pass walks the list).
 cudaError_t hip_build_fine(const float *pos, const float *w, int64_t N, double L, int n_c, int g, int64_t p0, int64_t p1,
                            const PmFineBuf &b, double *S1, double *wabs, int *err, cudaStream_t st);
 
@@ -67,7 +69,6 @@ struct PmPairCat {
     float R0, dc;
     double L, cs;          // box side, coarse cell side
     const double *wabs;    // sum |w|: sets the fixed-point unit
-    const int *err;        // the build's error word: a catalog it rejected is passed over
     double *G;             // [n_ell][Q][n_c S] FP64 totals (zero before the launch)
     unsigned long long *npairs;
     // work items: blocks of 32 sorted particles x n_col groups of neighbour columns x
