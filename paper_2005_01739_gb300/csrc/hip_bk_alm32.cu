@@ -13,7 +13,7 @@
 // their loads are already packed and the constants stored twice: the FP32 pipe does
 // the same work per operation, but at half the issue slots, which is what the
 // scalar form ran out of (251 warp instructions per pair at 75 % of the issue slots;
-// now 139, the FP32 pipe 52 % active; 5e5 data and 1.5e6 random primaries: 73.8 ->
+// now 137, the FP32 pipe 52 % active; 5e5 data and 1.5e6 random primaries: 73.8 ->
 // 46 ms).  The operations and their order are those of hip_F_b32.  The edge sums
 // stay one running sum each: two partial sums per edge would halve their
 // instructions too, but round differently (5e-8 of B).  Two packed pairs at a time
